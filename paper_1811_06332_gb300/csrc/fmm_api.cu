@@ -63,7 +63,7 @@ struct fmm_plan {
     float* Rpart = nullptr;              // level 5's source-class group sums of those products
     int64_t rpart_cap = 0;               // floats in Rpart
     int tc_source = 0;                   // 0 default, 1 autotuned, 2 from the cache, 3 set by the caller
-    cudaGraphExec_t ugexec = nullptr;    // uniform plans with use_graph: the captured step
+    cudaGraphExec_t ugexec = nullptr;    // uniform plans with use_graph: the captured step (dropped with the tree's buffers)
     const void* ugkey[11] = {nullptr};   // what the captured step depends on
     int tc_ncand = 0;
     int tc_cand[8][4];                   // autotuner candidates: kernel, cw, niss, microseconds
@@ -500,6 +500,8 @@ int fmm_direct(int64_t n, const double* x, const double* y, const double* z, con
 // plan
 // ---------------------------------------------------------------------------
 static void free_tree(fmm_plan* pl) {
+    // the captured step holds the addresses of the buffers freed here
+    if (pl->ugexec) { cudaGraphExecDestroy(pl->ugexec); pl->ugexec = nullptr; }
     cudaFree(pl->xs); cudaFree(pl->ys); cudaFree(pl->zs); cudaFree(pl->qs);
     cudaFree(pl->perm); cudaFree(pl->start); cudaFree(pl->scratch);
     cudaFree(pl->Mbuf); cudaFree(pl->Lbuf); cudaFree(pl->M32); cudaFree(pl->Mbf); cudaFree(pl->pos32);
@@ -737,7 +739,6 @@ void fmm_destroy(fmm_plan* pl) {
     ad_free(pl->ad);
     free_tree(pl);
     cudaFree(pl->W); cudaFree(pl->V); cudaFree(pl->Dtab); cudaFree(pl->stage);
-    if (pl->ugexec) cudaGraphExecDestroy(pl->ugexec);
     cudaFree(pl->Kbf); cudaFree(pl->Kgen); cudaFree(pl->derr); cudaFree(pl->W32); cudaFree(pl->V32); cudaFree(pl->mlp_dev);
     cudaFree(pl->part32);
     cudaFree(pl->Mrest); cudaFree(pl->Krest); cudaFree(pl->Rpart);
