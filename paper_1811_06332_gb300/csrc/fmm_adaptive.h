@@ -87,7 +87,7 @@ struct AdState {
     // captured operator sequence
     cudaGraphExec_t gexec = nullptr;
     bool graph_ok = false;
-    const void* graph_key[11] = {nullptr};
+    std::vector<uint64_t> graph_key;   // all that it holds by value (fmm_evaluate)
 };
 
 void ad_free(AdState* a);

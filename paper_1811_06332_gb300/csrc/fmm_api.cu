@@ -1064,18 +1064,17 @@ int fmm_evaluate(fmm_plan* pl, int64_t n, const double* x, const double* y, cons
         // replay the captured operator sequence while the tree keeps its
         // sizes and buffers; capture it again otherwise
         AdState* A = pl->ad;
-        // what the captured launches hold by value: level ranges, root side and
-        // the unit of the integer centres, the near field's segments
-        uint64_t lv = 1469598103934665603ull, sd = 0;
-        for (int v : A->lvl) lv = (lv ^ (uint64_t)v) * 1099511628211ull;
-        memcpy(&sd, &A->side, 8);
-        const void* key[11] = {A->M, pot, ax, (const void*)(intptr_t)A->gen, (const void*)(intptr_t)A->nn,
-                              (const void*)(uintptr_t)lv, (const void*)(uintptr_t)sd,
-                              (const void*)(intptr_t)(((int64_t)A->pseg << 1) | (A->pslots > 0)),
-                              (const void*)(intptr_t)(((int64_t)A->ntarg << 32) ^ A->nleaf ^ (A->nm2l * 7919LL)),
-                              (const void*)(intptr_t)((A->orders_fixed ? 1 : 0) | (pl->mlp_set ? 2 : 0)),
-                              (const void*)(intptr_t)A->m2l_blocks};
-        if (!A->gexec || memcmp(key, A->graph_key, sizeof key) != 0) {
+        // all that the captured launches hold: the four output arrays, the plan's
+        // buffers (gen counts their moves) and, by value, the particle, node and
+        // list counts, the root side (which gives the unit of the integer centres),
+        // the near field's segments, the orders' source and threshold, the level ranges
+        auto bits = [](auto v) { uint64_t u = 0; memcpy(&u, &v, sizeof v); return u; };
+        std::vector<uint64_t> key = {bits(pot), bits(ax), bits(ay), bits(az), bits(A->gen), bits(A->n), bits(A->nn),
+                                     bits(A->ntarg), bits(A->nleaf), bits(A->nm2l), bits(A->side), bits(A->pseg),
+                                     A->pslots > 0, A->orders_fixed, pl->mlp_set, bits(pl->log10_kappa),
+                                     bits(A->m2l_blocks)};
+        for (int v : A->lvl) key.push_back(bits(v));
+        if (!A->gexec || key != A->graph_key) {
             if (A->gexec) { cudaGraphExecDestroy(A->gexec); A->gexec = nullptr; }
             cudaGraph_t g = nullptr;
             CK(cudaStreamBeginCapture(S(stream), cudaStreamCaptureModeThreadLocal));
@@ -1089,7 +1088,7 @@ int fmm_evaluate(fmm_plan* pl, int64_t n, const double* x, const double* y, cons
             const cudaError_t ie = cudaGraphInstantiate(&A->gexec, g, 0);
             cudaGraphDestroy(g);
             if (ie != cudaSuccess) FAIL(FMM_ERR_CUDA, "graph instantiation failed: %s", cudaGetErrorString(ie));
-            memcpy(A->graph_key, key, sizeof key);
+            A->graph_key = key;
         }
         CK(cudaGraphLaunch(A->gexec, S(stream)));
         return FMM_OK;

@@ -58,3 +58,60 @@ def test_host_entry_with_changing_sizes():
         assert plan.stats()["graph"] == held
         assert np.array_equal(out, eager(X, **cfg).cpu().numpy())
     plan.close()
+
+
+def adaptive_outputs(plan, stream, X, out):
+    for a in out:
+        a.fill_(7.0)
+    stream.wait_stream(torch.cuda.current_stream())
+    plan.fmm_evaluate(*X, *out, stream=stream)
+    stream.synchronize()
+
+
+@pytest.mark.parametrize("swap", [0, 1, 2, 3])
+def test_adaptive_replay_writes_the_arrays_it_is_given(swap):
+    cfg = dict(p=4, basis=0, prec=F.FP32, adaptive=True, max_leaf=32, theta=0.6)
+    X = arrays(5000, 3)
+    plan, stream = F.Plan(use_graph=True, **cfg), torch.cuda.Stream()
+    old = torch.empty(4, 5000, dtype=torch.float64, device="cuda")
+    for _ in range(3):
+        adaptive_outputs(plan, stream, X, old)
+    assert plan.stats()["graph"] == 1
+    ref, new = old.clone(), torch.empty_like(old)
+    given = list(old)
+    given[swap] = new[swap]   # one of the four is another array; the old ones stay allocated
+    old[swap] = 3.0
+    adaptive_outputs(plan, stream, X, given)
+    assert torch.equal(torch.stack(given), ref)
+    assert torch.all(old[swap] == 3.0)
+    plan.close()
+
+
+def test_learned_replay_follows_a_new_threshold():
+    """The model's threshold shift (blob[6]) is held by value in the captured launches."""
+    X = arrays(6000, 4)
+    cfg = dict(p=6, basis=0, prec=F.FP32, adaptive=True, max_leaf=32, theta=0.6, learned_p=True, target_rel_err=1e-4)
+    blob = np.zeros(F.MLP_NBLOB, dtype=np.float32)
+    blob[:8] = [6332.0, 2.0, 12, 64, 9, 2.0, 0.0, 0.0]
+    blob[20:32] = 1.0
+    blob[-9:] = -np.arange(2, 11)   # the same log10 errors for every pair: order q gives 10^-q
+    low = blob.copy()
+    low[6] = 2.0                    # errors 100 times as large are accepted
+    plan, stream = F.Plan(use_graph=True, **cfg), torch.cuda.Stream()
+    out = torch.empty(4, 6000, dtype=torch.float64, device="cuda")
+    got = []
+    for b in (blob, low):
+        plan.set_mlp(b)
+        for _ in range(3):
+            adaptive_outputs(plan, stream, X, out)
+        got.append((out.clone(), plan.stats()["pairs_per_order"]))
+    plan.close()
+    for b, (res, per) in zip((blob, low), got):
+        ep = F.Plan(**cfg)
+        ep.set_mlp(b)
+        pot, acc = ep.evaluate(*X)
+        torch.cuda.synchronize()
+        assert per == ep.stats()["pairs_per_order"]
+        assert torch.equal(res, torch.cat([pot[None], acc]))
+        ep.close()
+    assert got[0][1] != got[1][1]
