@@ -342,10 +342,14 @@ __device__ __forceinline__ void mlp_outer(const float* g, const float* x, float 
 // Forward and backward of the batch rows order[0..nb); loss: mean over the
 // batch and the 9 outputs of (y - t)^2.  Block b takes the groups b, b + gridDim.x,
 // ..., and writes its gradient (blob order) to part[b] and its loss to lossp[b].
+// prm is what the step before writes while this kernel may already run: it is no
+// __restrict__ pointer, so that its loads are ordinary ones, which the wait orders
+// (a read-only load takes its data as unchanged for the whole kernel, and may be
+// moved ahead of the wait); likewise part and lossp in k_mlp_update.
 __global__ void __launch_bounds__(256)
 k_mlp_step(int nb, int64_t n, const int* __restrict__ order, const float* __restrict__ feat,
-           const float* __restrict__ lab, const float* __restrict__ prm, const float* __restrict__ mu,
-           const float* __restrict__ sd, float* __restrict__ part, float* __restrict__ lossp) {
+           const float* __restrict__ lab, const float* prm, const float* __restrict__ mu,
+           const float* __restrict__ sd, float* part, float* lossp) {
     extern __shared__ __align__(16) unsigned char raw[];
     MlpSmem& S = *reinterpret_cast<MlpSmem*>(raw);
     const int tid = threadIdx.x, s = tid & 7, u0 = tid >> 3;
@@ -486,9 +490,8 @@ static_assert(FMM_MLP_NF == 12 && FMM_MLP_NOUT == 9 && FMM_MLP_H == 64, "thread 
 // m = b1 m + (1-b1) g, v = b2 v + (1-b2) g^2,
 // theta -= lr (m/(1-b1^t)) / (sqrt(v/(1-b2^t)) + eps); without m, g to grad.
 __global__ void __launch_bounds__(256)
-k_mlp_update(int nblk, const float* __restrict__ part, const float* __restrict__ lossp, float* __restrict__ loss,
-             float* __restrict__ grad, float* __restrict__ prm, float* __restrict__ m, float* __restrict__ v, float lr,
-             float b1, float b2, float eps, float c1, float c2) {
+k_mlp_update(int nblk, const float* part, const float* lossp, float* loss, float* grad, float* prm, float* m, float* v,
+             float lr, float b1, float b2, float eps, float c1, float c2) {
     __shared__ float sg[8][32];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, t = blockIdx.x * 32 + lane;
     float a = 0.f, m0 = 0.f, v0 = 0.f, p0 = 0.f;
