@@ -791,7 +791,8 @@ int fmm_build_tree(fmm_plan* pl, int64_t n, const double* x, const double* y, co
         }
         const int deep = rf_deep(pl);
         if (deep >= 2) {
-            const int64_t pe = rf_part_elems(bL(pl) ? nt_of(pl->cfg.p) : ns_of(pl->cfg.p), deep, RF_MOST);
+            const int64_t pe = rf_part_elems(bL(pl) ? nt_of(pl->cfg.p) : ns_of(pl->cfg.p), deep, RF_MOST,
+                                              pl->cfg.prec != FMM_FP64);
             const size_t fb = (size_t)rf_fold_elems(pl->cfg.p, 2, deep) * (pl->cfg.prec == FMM_FP64 ? 8 : 4);
             if (cudaMalloc(&pl->mfold, fb) != cudaSuccess ||
                 (pe > 0 && cudaMalloc(&pl->mpart, (size_t)pe * (pl->L32 ? 4 : 8)) != cudaSuccess)) {

@@ -107,7 +107,7 @@ struct RfLevel { int l, g, end; int64_t F, L, part; };   // level, shares per ce
 struct RfLevels { int n; RfLevel v[FMM_PMAX]; };
 int64_t rf_fold_elems(int p, int lo, int hi);
 constexpr int RF_MOST = 56;   // shares of the 56 orbits at most
-int64_t rf_part_elems(int nrow, int deep, int most);
+int64_t rf_part_elems(int nrow, int deep, int most, bool f32);
 int launch_m2l_reflect(int out, int p, int symM, int symL, int lo, int hi, int deep, const int64_t* lvl_off,
                        const double* M, const float* M32, const double* Dtab, void* F, void* Lt, void* part, int most,
                        cudaStream_t s);

@@ -37,7 +37,15 @@ static int64_t rf_warps(int l) {   // warps of 32 cells of one class
 // all levels together give about 24 warps per SM (three times what an SM holds
 // in FP64 at p = 8: the last shares are short), at most `most`.  It does not
 // depend on the levels of one call: a call per level sums as one call does.
-static int rf_shares(int l, int deep, int sms, int most) {
+// FP32 (f32): an orbit per share on levels 2 and 3.  Most of the far potential
+// comes from them, and a thread's sum over many orbits rounds each product at
+// the size of the whole sum (k_rf_sum adds the shares without that).  Rounding
+// error of the far potential, depth 5, p = 4 / 6 / 8 traceless, rms: 1.91 / 2.33 /
+// 2.54e-7 with the rule below on every level, 1.75 / 2.15 / 2.30e-7 so (1.80 /
+// 2.21 / 2.40e-7 with offset by offset sums); the M2L 113 / 273 / 691 -> 121 / 265
+// / 650 us at 1,000,003 particles.
+static int rf_shares(int l, int deep, int sms, int most, bool f32) {
+    if (f32 && l <= 3) return most;
     int64_t tot = 0;
     for (int k = 2; k <= deep; ++k) tot += rf_warps(k);
     if (rf_warps(l) >= 32 * (int64_t)sms) return 1;
@@ -45,7 +53,7 @@ static int rf_shares(int l, int deep, int sms, int most) {
 }
 
 // layout of levels lo..hi; returns the number of units (warps' shares)
-static int rf_levels(int nrow, int lo, int hi, int deep, const int64_t* lvl_off, int p, int sms, int most,
+static int rf_levels(int nrow, int lo, int hi, int deep, const int64_t* lvl_off, int p, int sms, int most, bool f32,
                      RfLevels& lv) {
     int64_t F = 0, part = 0;
     int unit = 0;
@@ -53,7 +61,7 @@ static int rf_levels(int nrow, int lo, int hi, int deep, const int64_t* lvl_off,
     for (int l = lo; l <= hi; ++l) {
         RfLevel& v = lv.v[lv.n++];
         v.l = l;
-        v.g = rf_shares(l, deep, sms, most);
+        v.g = rf_shares(l, deep, sms, most, f32);
         unit += (int)rf_warps(l) * v.g;
         v.end = unit;
         v.F = F;
@@ -72,10 +80,10 @@ static int rf_sms() {
     return sms > 0 ? sms : 1;
 }
 
-int64_t rf_part_elems(int nrow, int deep, int most) {
+int64_t rf_part_elems(int nrow, int deep, int most, bool f32) {
     int64_t n = 0;
     for (int l = 2; l <= deep; ++l) {
-        const int g = rf_shares(l, deep, rf_sms(), most);
+        const int g = rf_shares(l, deep, rf_sms(), most, f32);
         if (g > 1) n += (int64_t)g * nrow << (3 * l);
     }
     return n;
@@ -112,7 +120,9 @@ k_rf_fold(int sym, int nc, int nt, int lo, int hi, const TI* __restrict__ M, T* 
     F[(int64_t)t * (ncell + RF_PAD_CELLS) + i] = v;
 }
 
-// partial sums of the split levels, added in group order
+// Partial sums of the split levels, added in group order; FP32 sums carry their
+// rounding errors along (the exact error of each addition), so that the result
+// is rounded once whatever the number of shares.
 template <typename OT>
 __global__ void __launch_bounds__(256)
 k_rf_sum(RfLevels lv, int nrow, const OT* __restrict__ part, OT* __restrict__ Lt) {
@@ -123,9 +133,16 @@ k_rf_sum(RfLevels lv, int nrow, const OT* __restrict__ part, OT* __restrict__ Lt
         const int64_t m = (int64_t)nrow << (3 * v.l);
         if (i >= m) { i -= m; continue; }
         const OT* p = part + v.part + i;
-        OT s = p[0];
-        for (int g = 1; g < v.g; ++g) s += p[(int64_t)g * m];
-        Lt[v.L + i] = s;
+        OT s = p[0], c = OT(0);
+        for (int g = 1; g < v.g; ++g) {
+            const OT a = p[(int64_t)g * m], t = s + a;
+            if constexpr (sizeof(OT) == 4) {
+                const OT u = t - s;
+                c += (s - (t - u)) + (a - u);
+            }
+            s = t;
+        }
+        Lt[v.L + i] = s + c;
         return;
     }
 }
@@ -135,7 +152,7 @@ k_rf_sum(RfLevels lv, int nrow, const OT* __restrict__ part, OT* __restrict__ Lt
 // symM, symL: symmetric storage of the multipoles and the locals.  M: the
 // multipoles from level lo on (M32 instead where given: their FP32 copy), Lt:
 // the locals from level lo on, lvl_off: the levels' offsets.  F: rf_fold_elems
-// elements, part: rf_part_elems with the same `most` (shares at most, 1..56).
+// elements, part: rf_part_elems with the same `most` (shares at most, 1..56) and f32 = (out != 0).
 // Returns the launches made.
 int launch_m2l_reflect(int out, int p, int symM, int symL, int lo, int hi, int deep, const int64_t* lvl_off,
                        const double* M, const float* M32, const double* Dtab, void* F, void* Lt, void* part, int most,
@@ -143,7 +160,7 @@ int launch_m2l_reflect(int out, int p, int symM, int symL, int lo, int hi, int d
     if (lo > hi) return 0;
     const int nt = nt_of(p), ncM = symM ? ns_of(p) : nt, nrow = symL ? ns_of(p) : nt;
     RfLevels lv;
-    const int units = rf_levels(nrow, lo, hi, deep, lvl_off, p, rf_sms(), most, lv);
+    const int units = rf_levels(nrow, lo, hi, deep, lvl_off, p, rf_sms(), most, out != 0, lv);
     int64_t cells = 0, sums = 0;
     for (int l = lo; l <= hi; ++l) cells += ((int64_t)1 << (3 * l)) + RF_PAD_CELLS;
     for (int i = 0; i < lv.n; ++i)
