@@ -41,7 +41,7 @@ static int64_t rf_warps(int l) {   // warps of 32 cells of one class
 // comes from them, and a thread's sum over many orbits rounds each product at
 // the size of the whole sum (k_rf_sum adds the shares without that).  Rounding
 // error of the far potential, depth 5, p = 4 / 6 / 8 traceless, rms: 1.91 / 2.33 /
-// 2.54e-7 with the rule below on every level, 1.75 / 2.15 / 2.30e-7 so (1.80 /
+// 2.54e-7 with the rule below on every level, 1.74 / 2.15 / 2.31e-7 so (1.80 /
 // 2.21 / 2.40e-7 with offset by offset sums); the M2L 113 / 273 / 691 -> 121 / 265
 // / 650 us at 1,000,003 particles.
 static int rf_shares(int l, int deep, int sms, int most, bool f32) {
