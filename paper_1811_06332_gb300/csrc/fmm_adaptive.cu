@@ -616,7 +616,7 @@ int ad_leaf_keys(int nn, int n, const int* nchild, const int* nb, uint32_t* key,
 //   c_(a,b,c) = sum_{i <= a/2, k <= b/2} (-1)^(i+k) C(i+k, i) M_m / m!,
 //   m = (a - 2i, b - 2k, c + 2(i + k)),  c = 0 or 1
 // (traceless storage: with the dependent M_m written out in the stored ones),
-// in T, rows of ldm, padded with zeros.  Done once per node here instead of once
+// summed in FP64 and rounded once to T, rows of ldm, padded with zeros.  Done once per node here instead of once
 // per pair: a row is nt(p) components instead of ns(p) (p = 6: 49 instead of 84),
 // which the M2L kernels gather per pair.  The terms of a component are a table
 // (generated, the same for every order), copied to shared memory once per
@@ -625,25 +625,25 @@ constexpr int FOLD_ROWS = 64;
 template <typename T>
 __global__ void __launch_bounds__(256)
 k_fold(int64_t rows, int p, int basis, int ldm, const double* __restrict__ M, T* __restrict__ F) {
-    __shared__ T sC[FMM_FOLD_MAX];
+    __shared__ double sC[FMM_FOLD_MAX];
     __shared__ unsigned short sIdx[FMM_FOLD_MAX], sOff[FMM_NT_MAX + 1];
     const int nt = nt_of(p), nc = ncoef_of(p, basis);
     const unsigned short* off = basis ? d_fold_off1 : d_fold_off0;
     const unsigned short* idx = basis ? d_fold_idx1 : d_fold_idx0;
     const double* cf = basis ? d_fold_c1 : d_fold_c0;
     for (int t = threadIdx.x; t <= nt; t += 256) sOff[t] = off[t];
-    for (int k = threadIdx.x; k < off[nt]; k += 256) { sIdx[k] = idx[k]; sC[k] = T(cf[k]); }
+    for (int k = threadIdx.x; k < off[nt]; k += 256) { sIdx[k] = idx[k]; sC[k] = cf[k]; }
     __syncthreads();
     const int64_t r0 = (int64_t)blockIdx.x * FOLD_ROWS;
     const int cnt = (int)(rows - r0 < FOLD_ROWS ? rows - r0 : FOLD_ROWS) * ldm;
     for (int i = threadIdx.x; i < cnt; i += 256) {
         const int r = i / ldm, t = i - r * ldm;
-        T v = T(0);
+        double v = 0.0;
         if (t < nt) {
             const double* Mr = M + (r0 + r) * nc;
-            for (int k = sOff[t]; k < sOff[t + 1]; ++k) v = fma(sC[k], T(Mr[sIdx[k]]), v);
+            for (int k = sOff[t]; k < sOff[t + 1]; ++k) v = fma(sC[k], Mr[sIdx[k]], v);
         }
-        F[r0 * ldm + i] = v;
+        F[r0 * ldm + i] = T(v);
     }
 }
 int ad_fold(int prec, int64_t rows, int p, int basis, int ldm, const double* M, void* F, cudaStream_t s) {
