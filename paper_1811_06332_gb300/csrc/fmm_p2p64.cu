@@ -90,7 +90,7 @@ __device__ __forceinline__ void p2p64_batch(int lane, int grp, int G, bool act, 
             for (int j = 0; j < NT; ++j) {
                 const double dx = a.x - xt[j], dy = a.y - yt[j], dz = b.x - zt[j];
                 const double ir = rsqrt_or0(fma(dx, dx, fma(dy, dy, dz * dz)));   // self, coincident: 0
-                const double qir = b.y * ir, w = qir * (ir * ir);
+                const double qir = b.y * ir, w = qir * ir * ir;   // ir * ir alone may overflow
                 ph[j] += qir;
                 gx[j] = fma(w, dx, gx[j]);
                 gy[j] = fma(w, dy, gy[j]);
