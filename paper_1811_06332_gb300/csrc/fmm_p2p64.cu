@@ -213,7 +213,9 @@ k_p2p64_uniform(int depth, int64_t nleaf, const int* __restrict__ start, P2P64In
 // targets' in shared memory (a copy per group of tn lanes).  The sources' sums go
 // to a slot of their own per direction, slots[13][4][n], which k_p2p64_back adds
 // to the particles afterwards: no two warps write one word, and the sums run
-// in a fixed order.  The leaf's own pairs take the one-sided form.
+// in a fixed order.  The leaf's own pairs take the one-sided form.  (1/r)^3 does
+// not overflow: points of the unit cube in different leaves differ by at least
+// 2^-63 along some axis, and points outside it by as much.
 // Measured, 524,288 particles at depth 5: 8.2 -> 5.4 ms; 120,011 at depth 4: 3.2 ->
 // 2.2 ms; but 4,096 at depth 3: 84 -> 99 us (see launch_p2p64).
 // ---------------------------------------------------------------------------

@@ -98,12 +98,14 @@ __device__ __forceinline__ void rf_orbit(int u, int& a, int& b, int& c) {
     a = o & 3; b = (o >> 2) & 3; c = o >> 4;
 }
 
-// entry K of the warp's D components at shared address sa
+// Entry K of the warp's D components at shared address sa.  volatile: the
+// compiler knows nothing of the memory that is read, and a plain asm could be
+// moved past the barriers and stores of the next orbit's rf_stage.
 template <typename T, int K>
 __device__ __forceinline__ T rf_lds(unsigned sa) {
     T v;
-    if constexpr (sizeof(T) == 4) asm("ld.shared.f32 %0, [%1+%2];" : "=f"(v) : "r"(sa), "n"(4 * K));
-    else asm("ld.shared.f64 %0, [%1+%2];" : "=d"(v) : "r"(sa), "n"(8 * K));
+    if constexpr (sizeof(T) == 4) asm volatile("ld.shared.f32 %0, [%1+%2];" : "=f"(v) : "r"(sa), "n"(4 * K));
+    else asm volatile("ld.shared.f64 %0, [%1+%2];" : "=d"(v) : "r"(sa), "n"(8 * K));
     return v;
 }
 
