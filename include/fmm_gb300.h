@@ -194,7 +194,12 @@ int fmm_l2l(fmm_plan* plan, void* stream);
  * caller order) with the far-field potential and acceleration. */
 int fmm_l2p(fmm_plan* plan, double* pot, double* ax, double* ay, double* az, void* stream);
 /* Near field (App. C direct sum over adjacent leaves, self excluded):
- * ADDS into pot, ax, ay, az (device, length n, caller order). */
+ * ADDS into pot, ax, ay, az (device, length n, caller order).
+ * FMM_FP64 on a uniform octree: from about 27 n^2 / 8^depth = 4e6 pairs on, up to
+ * 2^24 particles, every pair of particles of two leaves is evaluated once, with
+ * 416 bytes per particle of plan storage; where that could not be allocated
+ * (fmm_plan_stats, out[19]) every pair is evaluated from both sides, to the same
+ * accuracy but with other roundings, as it is below and above these sizes. */
 int fmm_p2p(fmm_plan* plan, double* pot, double* ax, double* ay, double* az, void* stream);
 /* L2P followed by P2P in one pass: writes (does not add) pot and acc of
  * every particle with the far field of its leaf's local expansion and the
@@ -366,10 +371,11 @@ int fmm_evaluate_noalloc(int p, int basis, int depth, int64_t n, const double* x
                          double* az, void* stream);
 
 /* Sizes of the plan's tree and lists after fmm_build_tree, written to
- * out[0..min(nout,19)): number of cells, leaves, M2L pairs, P2P (leaf) pairs,
+ * out[0..min(nout,20)): number of cells, leaves, M2L pairs, P2P (leaf) pairs,
  * M2L target cells, autotuned M2L blocks per SM (0 before the first M2L),
  * tree levels, 1 when a captured operator graph is held, then (learned_p
- * plans, after an M2L) the number of M2L pairs at each order 0..10.  For
+ * plans, after an M2L) the number of M2L pairs at each order 0..10, and 1 when
+ * the FP64 near field of a uniform tree evaluates every pair once (fmm_p2p).  For
  * uniform trees the list entries are 0 (the lists are implicit). */
 int fmm_plan_stats(const fmm_plan* plan, int64_t* out, int nout);
 

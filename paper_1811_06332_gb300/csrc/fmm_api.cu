@@ -355,7 +355,7 @@ int fmm_tune_cache_put(const char* path, const char* key, const int* vals, doubl
 
 int fmm_plan_stats(const fmm_plan* pl, int64_t* out, int nout) {
     if (!pl || !out || nout < 0) return fail_plan(nullptr, FMM_ERR_ARG, "null plan or output");
-    int64_t v[19] = {0};
+    int64_t v[20] = {0};
     if (pl->ad && pl->cfg.learned_p && nout > 8 && pl->built)
         ad_order_counts(pl->ad, pl->cfg.p, v + 8, 0);
     if (pl->ad) {
@@ -368,8 +368,9 @@ int fmm_plan_stats(const fmm_plan* pl, int64_t* out, int nout) {
         for (int l = 0; l <= pl->depth; ++l) cells += (int64_t)1 << (3 * l);
         v[0] = cells; v[1] = pl->nleaf; v[6] = pl->depth + 1;
         v[7] = pl->ugexec ? 1 : 0;
+        v[19] = pl->pslots ? 1 : 0;
     }
-    for (int k = 0; k < nout && k < 19; ++k) out[k] = v[k];
+    for (int k = 0; k < nout && k < 20; ++k) out[k] = v[k];
     return FMM_OK;
 }
 
@@ -801,10 +802,10 @@ int fmm_build_tree(fmm_plan* pl, int64_t n, const double* x, const double* y, co
                 FAIL(FMM_ERR_OOM, "allocating tree storage for n=%lld failed", (long long)n);
             }
         }
-        // the near field's mutual form takes 416 bytes per particle; without them (or
-        // past 2^24 particles) the one-sided form runs
-        if (pl->cfg.prec == FMM_FP64 && n > 0 && n <= ((int64_t)1 << 24) &&
-            cudaMalloc(&pl->pslots, (size_t)p2p64_slot_bytes(n)) != cudaSuccess) {
+        // the near field's mutual form takes 416 bytes per particle, where it is
+        // used; without them the one-sided form runs (its sums round differently)
+        const int64_t sb = pl->cfg.prec == FMM_FP64 && n > 0 ? p2p64_slot_bytes(n, pl->nleaf) : 0;
+        if (sb > 0 && cudaMalloc(&pl->pslots, (size_t)sb) != cudaSuccess) {
             cudaGetLastError();
             pl->pslots = nullptr;
         }

@@ -97,7 +97,7 @@ int launch_l2p_leaf2(int prec, int p, int basis, int depth, int64_t nleaf, const
                      const float4* pos32 = nullptr,
                      const float* Lt32 = nullptr);
 // fmm_p2p64.cu: FP64 near field of the uniform octree
-int64_t p2p64_slot_bytes(int64_t n);   // of the mutual form's sums per direction
+int64_t p2p64_slot_bytes(int64_t n, int64_t nleaf);   // of the mutual form's sums per direction; 0: one-sided
 int launch_p2p64(int depth, int64_t nleaf, const int* start, const double* xs, const double* ys, const double* zs,
                  const double* qs, const int* perm, double* pot, double* ax, double* ay, double* az, double* slots,
                  int64_t n, cudaStream_t s);

@@ -388,12 +388,16 @@ k_p2p64_back(int depth, int64_t nleaf, const int* __restrict__ start, const int*
     }
 }
 
-int64_t p2p64_slot_bytes(int64_t n) { return P2P64_DIRS * 4 * 8 * n; }
+// Bytes of slots for the mutual form where it is the faster one, else 0: from 4
+// million pairs, about 27 n^2 / nleaf, on; below, the time is the latency of a leaf's
+// chain and a second launch (one-sided against mutual: 0.9 million pairs 84 and 99
+// us; 95 million 3.2 and 2.2 ms).  Up to 2^24 particles (7 GB of slots).
+int64_t p2p64_slot_bytes(int64_t n, int64_t nleaf) {
+    const bool mutual = n <= ((int64_t)1 << 24) && 27.0 * (double)n * (double)n / (double)nleaf >= 4e6;
+    return mutual ? P2P64_DIRS * 4 * 8 * n : 0;
+}
 
-// The mutual form where slots (p2p64_slot_bytes(n), or null) are given and the
-// pairs, about 27 n^2 / nleaf, are 4 million or more: below, the time is the
-// latency of a leaf's chain and a second launch, and the one-sided form wins
-// (0.9 million pairs: 84 against 99 us; 95 million: 3.2 against 2.2 ms).
+// The mutual form where slots (p2p64_slot_bytes) are given, else the one-sided.
 int launch_p2p64(int depth, int64_t nleaf, const int* start, const double* xs, const double* ys, const double* zs,
                  const double* qs, const int* perm, double* pot, double* ax, double* ay, double* az, double* slots,
                  int64_t n, cudaStream_t s) {
@@ -404,7 +408,7 @@ int launch_p2p64(int depth, int64_t nleaf, const int* start, const double* xs, c
     // are 27 warps per SM, and the last, fullest leaf sets the time
     const bool four = nleaf <= 4096;
     const unsigned g = (unsigned)(four ? nleaf : (nleaf + 3) / 4);
-    if (slots && 27.0 * (double)n * (double)n / (double)nleaf >= 4e6) {
+    if (slots) {
         if (four) k_p2p64_mutual<4><<<g, 128, 0, s>>>(depth, nleaf, start, P, perm, O, slots, n);
         else k_p2p64_mutual<1><<<g, 128, 0, s>>>(depth, nleaf, start, P, perm, O, slots, n);
         k_p2p64_back<<<(unsigned)((nleaf + 3) / 4), 128, 0, s>>>(depth, nleaf, start, perm, O, slots, n);

@@ -337,11 +337,11 @@ class Plan:
         """Tree and list sizes (fmm_plan_stats); learned_p plans add the
         number of M2L pairs per order."""
         import numpy as np
-        v = np.zeros(19, dtype=np.int64)
-        self._c(lib().fmm_plan_stats(self.h, v.ctypes.data, 19))
+        v = np.zeros(20, dtype=np.int64)
+        self._c(lib().fmm_plan_stats(self.h, v.ctypes.data, 20))
         keys = ("cells", "leaves", "m2l_pairs", "p2p_pairs", "m2l_targets", "m2l_blocks_per_sm", "levels",
                 "graph")
-        out = dict(zip(keys, v[:8].tolist()))
+        out = dict(zip(keys, v[:8].tolist()), p2p_mutual=int(v[19]))
         if self.cfg.learned_p:
             out["pairs_per_order"] = v[8:8 + self.cfg.p + 1].tolist()
         return out
