@@ -128,16 +128,20 @@ __device__ __forceinline__ void p2p64_block(int lane, int t0, int tn, int k0, in
         p2p64_batch<NT>(lane, grp, G, act, xt, yt, zt, ph, gx, gy, gz, 32 * part, 32 * parts, total, sb, incl - cnt,
                         incl, P, sXY, sZQ);
     }
+    // the groups' sums, halving the groups (an order fixed by their number): a leaf
+    // of one particle has 32 of them
+    for (int h = G > 1 ? 1 << (31 - __clz(G - 1)) : 0; h; h >>= 1) {
+        const int src = min(31, lane + h * gw);
+        const bool take = grp + h < G && grp < h;
+#pragma unroll
+        for (int j = 0; j < NT; ++j) {
+            const double p0 = __shfl_sync(0xffffffffu, ph[j], src), x0 = __shfl_sync(0xffffffffu, gx[j], src),
+                         y0 = __shfl_sync(0xffffffffu, gy[j], src), z0 = __shfl_sync(0xffffffffu, gz[j], src);
+            if (take) { ph[j] += p0; gx[j] += x0; gy[j] += y0; gz[j] += z0; }
+        }
+    }
 #pragma unroll
     for (int j = 0; j < NT; ++j) {
-        const double p0 = ph[j], x0 = gx[j], y0 = gy[j], z0 = gz[j];
-        for (int g = 1; g < G; ++g) {   // the groups' sums in group order
-            const int src = min(31, tl + g * gw);
-            ph[j] += __shfl_sync(0xffffffffu, p0, src);
-            gx[j] += __shfl_sync(0xffffffffu, x0, src);
-            gy[j] += __shfl_sync(0xffffffffu, y0, src);
-            gz[j] += __shfl_sync(0xffffffffu, z0, src);
-        }
         const int k = tl + gw * j;
         if (grp == 0 && k < tn) put(k, ph[j], gx[j], gy[j], gz[j]);
     }
@@ -166,6 +170,7 @@ k_p2p64_uniform(int depth, int64_t nleaf, const int* __restrict__ start, P2P64In
     const int64_t c = (int64_t)blockIdx.x * (4 / WPL) + w / WPL;
     if (c >= nleaf) return;   // WPL 4: the whole block
     const int b = start[c], e = start[c + 1];
+    if (b == e) return;
     const int side = 1 << depth;
     int ix, iy, iz;
     cell_coords(depth, c, ix, iy, iz);
@@ -240,6 +245,7 @@ k_p2p64_mutual(int depth, int64_t nleaf, const int* __restrict__ start, P2P64In 
     const int64_t c = (int64_t)blockIdx.x * (4 / WPL) + w / WPL;
     if (c >= nleaf) return;   // WPL 4: the whole block
     const int b = start[c], e = start[c + 1];
+    if (b == e) return;
     int ix, iy, iz;
     cell_coords(depth, c, ix, iy, iz);
     // forward neighbours, one per lane
