@@ -389,8 +389,8 @@ static int m2l_launch(AdState* a, int p, int basis, int prec, int blocks, cudaSt
 int ad_run_m2l(AdState* a, int p, int basis, int prec, int sms, cudaStream_t s) {
     if (a->n == 0) return 0;
     cudaMemsetAsync(a->L, 0, (size_t)a->nn * a->nc * 8, s);
-    ad_fold(prec, a->nn, p, basis, ldf_of(prec, p), a->M, a->Mf, s);
     if (a->ntarg == 0) return 0;
+    ad_fold(prec, a->nn, p, basis, ldf_of(prec, p), a->M, a->Mf, s);
     if (a->m2l_blocks == 0) {
         // autotune the persistent grid on the first evaluation: candidates of
         // 1..4 blocks of 128 threads per SM, each timed once after a warm-up
@@ -478,8 +478,8 @@ int ad_run_m2l_orders(AdState* a, int p, int basis, int prec, int sms, const uns
                       cudaStream_t s) {
     if (a->n == 0) return 0;
     cudaMemsetAsync(a->L, 0, (size_t)a->nn * a->nc * 8, s);
-    ad_fold(prec, a->nn, p, basis, ldf_of(prec, p), a->M, a->Mf, s);
     if (a->nm2l == 0) return 0;
+    ad_fold(prec, a->nn, p, basis, ldf_of(prec, p), a->M, a->Mf, s);
     if (!a->orders_fixed) {
         ad_node_features(a, s);
         ad_far_estimate(a, s);
