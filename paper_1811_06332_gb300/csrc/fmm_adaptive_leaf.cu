@@ -79,7 +79,7 @@ k_ad_p2m(int basis, int nleaf, const int* __restrict__ leaf, const int* __restri
         for (int j = 0; j <= P; ++j) acc[kk][j] = T(0);
     int cnx[KC], cny[KC];
 #pragma unroll
-    for (int kk = 0; kk < KC; ++kk) p2m_column(lane + 32 * kk, cnx[kk], cny[kk]);
+    for (int kk = 0; kk < KC; ++kk) p2m_column<P>(lane + 32 * kk, cnx[kk], cny[kk]);
     double cx = 0.0, cy = 0.0, cz = 0.0;
     if (!pos32) { cx = zc[3 * c]; cy = zc[3 * c + 1]; cz = zc[3 * c + 2]; }
     const float hinv = pos32 ? (float)ldexp(1.0 / side, lev[c]) : 1.f;
@@ -160,9 +160,9 @@ k_ad_p2m(int basis, int nleaf, const int* __restrict__ leaf, const int* __restri
 // 8,388,608 particles, p = 6, FP32: 1.17 ms, the scattered writes of the caller's
 // order; the products no longer count.
 // ---------------------------------------------------------------------------
-template <int P, typename T, int WARPS>
+template <int P, typename T, int WARPS, int BASIS>
 __global__ void __launch_bounds__(WARPS * 32)
-k_ad_l2p(int basis, int nleaf, const int* __restrict__ leaf, const int* __restrict__ nb, const int* __restrict__ ne,
+k_ad_l2p(int nleaf, const int* __restrict__ leaf, const int* __restrict__ nb, const int* __restrict__ ne,
          const double* __restrict__ zc, const double* __restrict__ xs, const double* __restrict__ ys,
          const double* __restrict__ zs, const float4* __restrict__ pos32, const int* __restrict__ perm,
          const double* __restrict__ Ln, double* __restrict__ pot, double* __restrict__ ax, double* __restrict__ ay, double* __restrict__ az,
@@ -170,15 +170,21 @@ k_ad_l2p(int basis, int nleaf, const int* __restrict__ leaf, const int* __restri
     // FP32 form (pos32 given): scaled units of the leaf, Lt_n = L_n h^(|n|+1):
     // Phi = (1/h) sum_k (r/h)^k/k! Lt_k, grad = (1/h^2) sum_k (r/h)^k/k! Lt_{k+e_i}
     constexpr int NC = (P + 1) * (P + 2) * (P + 3) / 6, NT = (P + 1) * (P + 1);
-    __shared__ __align__(16) T sL[WARPS][leaf_col<P, T>(P + 1, 0)];
+    __shared__ __align__(16) T sL[WARPS][BASIS ? leaf_col<P, T>(P + 1, 0) : NC];
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int k = blockIdx.x * WARPS + w;
     if (k >= nleaf) return;
     const int c = leaf[k];
     const int b = nb[c], e = ne[c];
     if (b == e) return;
-    const double* Lc = Ln + (int64_t)c * (basis ? NT : NC);
-    local_columns<P, 32>(basis, lane, true, sL[w], [&](int t) { return T(Lc[t]); });
+    const double* Lc = Ln + (int64_t)c * (BASIS ? NT : NC);
+    if constexpr (BASIS) {
+        local_columns<P, 32>(1, lane, true, sL[w], [&](int t) { return T(Lc[t]); });
+    } else {
+        // symmetric storage stays in its order: a row is read by consecutive words
+        for (int s = lane; s < NC; s += 32) sL[w][s] = T(Lc[s]);
+        __syncwarp();
+    }
     double cx = 0.0, cy = 0.0, cz = 0.0;
     if (!pos32) { cx = zc[3 * c]; cy = zc[3 * c + 1]; cz = zc[3 * c + 2]; }
     const double hinv_d = pos32 ? ldexp(1.0 / side, lev[c]) : 1.0;
@@ -202,7 +208,7 @@ k_ad_l2p(int basis, int nleaf, const int* __restrict__ leaf, const int* __restri
             fz[kk] = fz[kk - 1] * rz * T(1.0 / kk);
         }
         T ph = 0, gx = 0, gy = 0, gz = 0;
-        l2p_all<P, T, 0>(sL[w], fx, fy, fz, ph, gx, gy, gz);
+        l2p_all<P, T, 0, BASIS != 0>(sL[w], fx, fy, fz, ph, gx, gy, gz);
         const int o = perm[a];
         pot[o] = -(double)ph * hinv_d;
         ax[o] = (double)gx * hinv_d * hinv_d;
@@ -431,10 +437,16 @@ int ad_l2p_leaf(int prec, int p, int basis, int nleaf, const int* leaf, const in
     if (nleaf <= 0) return 0;
     constexpr int W = 4;
     const unsigned g = (unsigned)((nleaf + W - 1) / W);
-#define C64(P) k_ad_l2p<P, double, W><<<g, W * 32, 0, s>>>(basis, nleaf, leaf, nb, ne, zc, xs, ys, zs, nullptr, \
-                                                            perm, Ln, pot, ax, ay, az, lev, side)
-#define C32(P) k_ad_l2p<P, float, W><<<g, W * 32, 0, s>>>(basis, nleaf, leaf, nb, ne, zc, xs, ys, zs, pos32, \
-                                                           perm, Ln, pot, ax, ay, az, lev, side)
+#define C64(P)                                                                                                       \
+    if (basis) k_ad_l2p<P, double, W, 1><<<g, W * 32, 0, s>>>(nleaf, leaf, nb, ne, zc, xs, ys, zs, nullptr, perm, Ln, \
+                                                              pot, ax, ay, az, lev, side);                             \
+    else k_ad_l2p<P, double, W, 0><<<g, W * 32, 0, s>>>(nleaf, leaf, nb, ne, zc, xs, ys, zs, nullptr, perm, Ln, pot,   \
+                                                        ax, ay, az, lev, side)
+#define C32(P)                                                                                                       \
+    if (basis) k_ad_l2p<P, float, W, 1><<<g, W * 32, 0, s>>>(nleaf, leaf, nb, ne, zc, xs, ys, zs, pos32, perm, Ln,     \
+                                                             pot, ax, ay, az, lev, side);                             \
+    else k_ad_l2p<P, float, W, 0><<<g, W * 32, 0, s>>>(nleaf, leaf, nb, ne, zc, xs, ys, zs, pos32, perm, Ln, pot, ax,  \
+                                                       ay, az, lev, side)
     if (prec == 0) { AD_P_SWITCH(p, C64) } else { AD_P_SWITCH(p, C32) }
 #undef C64
 #undef C32

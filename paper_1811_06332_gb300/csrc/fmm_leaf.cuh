@@ -10,9 +10,10 @@ namespace fmm {
 // p = 8 lanes 0..31 hold columns of 9 to 2 components and the 13 columns of the
 // second turn have at most 2, so that turn takes 2 products per particle instead
 // of the 9 of an order by nx, and the columns of a z power >= k are the first ones.
+template <int P>
 __device__ __forceinline__ void p2m_column(int c, int& nx, int& ny) {
     int s = 0;
-    while ((s + 1) * (s + 2) / 2 <= c) ++s;
+    while (s < P && (s + 1) * (s + 2) / 2 <= c) ++s;   // (past the last column: anything)
     ny = c - s * (s + 1) / 2;
     nx = s - ny;
 }
@@ -81,7 +82,7 @@ __device__ __forceinline__ void local_columns(int basis, int lane, bool valid, T
         o0[k] = ox[k] = oy[k] = 0;
         if (col < NCOL) {
             int nx, ny;
-            p2m_column(col, nx, ny);
+            p2m_column<P>(col, nx, ny);
             const int s = nx + ny;
             o0[k] = leaf_col<P, T>(s, ny);
             if (s + 2 <= P) {
@@ -93,7 +94,13 @@ __device__ __forceinline__ void local_columns(int basis, int lane, bool valid, T
                     Ls[o0[k]] = ld(s * s + ny);
                     if (s < P) Ls[o0[k] + 1] = ld((s + 1) * (s + 1) + s + 2 + ny);
                 } else {
-                    for (int z = 0; z <= P - s; ++z) Ls[o0[k] + z] = ld(pos_sym(nx, ny, z));
+                    T v[P + 1];   // all loads of the column in flight together
+#pragma unroll
+                    for (int z = 0; z <= P; ++z)
+                        if (z <= P - s) v[z] = ld(pos_sym(nx, ny, z));
+#pragma unroll
+                    for (int z = 0; z <= P; ++z)
+                        if (z <= P - s) Ls[o0[k] + z] = v[z];
                 }
             }
         }
@@ -121,13 +128,18 @@ __device__ __forceinline__ void local_columns(int basis, int lane, bool valid, T
 // point takes 2 products per component (at p = 8, 460 with the outer sums)
 // instead of the 4 of four separate sums (740) and a third of the shared reads.
 // ---------------------------------------------------------------------------
-template <int P, typename T, int KX, int KY>
+template <int P, typename T, int KX, int KY, bool COLS>
 __device__ __forceinline__ void l2p_row(const T* __restrict__ Ln, const T (&fy)[P + 1], const T (&fz)[P + 1],
                                         T& xp, T& xy, T& xz) {
     if constexpr (KY <= P - KX) {
         constexpr int LEN = P + 1 - KX - KY;
         T c[LEN];
-        load16<T, LEN>(Ln + leaf_col<P, T>(KX + KY, KY), c);
+        if constexpr (COLS) {
+            load16<T, LEN>(Ln + leaf_col<P, T>(KX + KY, KY), c);
+        } else {
+#pragma unroll
+            for (int z = 0; z < LEN; ++z) c[z] = Ln[pos_sym(KX, KY, z)];
+        }
         T y = T(0), yz = T(0);
 #pragma unroll
         for (int z = 0; z < LEN; ++z) {
@@ -137,20 +149,21 @@ __device__ __forceinline__ void l2p_row(const T* __restrict__ Ln, const T (&fy)[
         xp = fma(fy[KY], y, xp);
         if constexpr (KY > 0) xy = fma(fy[KY - 1], y, xy);
         if constexpr (LEN > 1) xz = fma(fy[KY], yz, xz);
-        l2p_row<P, T, KX, KY + 1>(Ln, fy, fz, xp, xy, xz);
+        l2p_row<P, T, KX, KY + 1, COLS>(Ln, fy, fz, xp, xy, xz);
     }
 }
-template <int P, typename T, int KX>
+// COLS: Ln as columns (local_columns); else in the order of symmetric storage
+template <int P, typename T, int KX, bool COLS = true>
 __device__ __forceinline__ void l2p_all(const T* __restrict__ Ln, const T (&fx)[P + 1], const T (&fy)[P + 1],
                                         const T (&fz)[P + 1], T& ph, T& gx, T& gy, T& gz) {
     if constexpr (KX <= P) {
         T xp = T(0), xy = T(0), xz = T(0);
-        l2p_row<P, T, KX, 0>(Ln, fy, fz, xp, xy, xz);
+        l2p_row<P, T, KX, 0, COLS>(Ln, fy, fz, xp, xy, xz);
         ph = fma(fx[KX], xp, ph);
         if constexpr (KX > 0) gx = fma(fx[KX - 1], xp, gx);
         gy = fma(fx[KX], xy, gy);
         gz = fma(fx[KX], xz, gz);
-        l2p_all<P, T, KX + 1>(Ln, fx, fy, fz, ph, gx, gy, gz);
+        l2p_all<P, T, KX + 1, COLS>(Ln, fx, fy, fz, ph, gx, gy, gz);
     }
 }
 

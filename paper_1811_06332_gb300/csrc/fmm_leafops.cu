@@ -58,7 +58,7 @@ k_p2m_leaf(int basis, int depth, int64_t nleaf, const int* __restrict__ start, c
         for (int j = 0; j <= P; ++j) acc[k][j] = T(0);
     int cnx[KC], cny[KC];
 #pragma unroll
-    for (int k = 0; k < KC; ++k) p2m_column(lane + 32 * k, cnx[k], cny[k]);
+    for (int k = 0; k < KC; ++k) p2m_column<P>(lane + 32 * k, cnx[k], cny[k]);
     for (int a0 = b; a0 < e; a0 += 32) {
         const int a = a0 + lane;
         __syncwarp();
@@ -88,6 +88,11 @@ k_p2m_leaf(int basis, int depth, int64_t nleaf, const int* __restrict__ start, c
             }
         }
         __syncwarp();
+        // two particles at a time where a lane has two columns (dense leaves are bound
+        // by the latency of a particle's products: 6,250 per leaf, p = 8, FP32 727 ->
+        // 467 us, one column per lane 437 -> 468; 4,194,304 in 262,144 leaves 404 -> 380)
+        constexpr int UN = sizeof(T) == 4 && KC > 1 ? 2 : 1;
+#pragma unroll UN
         for (int i = 0; i < cnt; ++i) {
             const T qa = sq[w][i];
             T zp[P + 1];   // the particle's z powers (same address across the warp)
