@@ -88,12 +88,7 @@ k_p2m_leaf(int basis, int depth, int64_t nleaf, const int* __restrict__ start, c
             }
         }
         __syncwarp();
-        // two particles at a time where a lane has two columns (dense leaves are bound
-        // by the latency of a particle's products: 6,250 per leaf, p = 8, FP32 727 ->
-        // 467 us, one column per lane 437 -> 468; 4,194,304 in 262,144 leaves 404 -> 380)
-        constexpr int UN = sizeof(T) == 4 && KC > 1 ? 2 : 1;
-#pragma unroll UN
-        for (int i = 0; i < cnt; ++i) {
+        auto particle = [&](int i) {
             const T qa = sq[w][i];
             T zp[P + 1];   // the particle's z powers (same address across the warp)
             if constexpr (sizeof(T) == 4) {
@@ -118,6 +113,15 @@ k_p2m_leaf(int basis, int depth, int64_t nleaf, const int* __restrict__ start, c
                             acc[k][j] = fma(wgt, zp[j], acc[k][j]);
                 }
             }
+        };
+        if constexpr (sizeof(T) == 4 && KC > 1) {
+            // two particles at a time where a lane has two columns: dense leaves are bound
+            // by the latency of a particle's products (50,000 particles in 8 leaves, p = 8,
+            // FP32 727 -> 467 us; 4,194,304 in 262,144 leaves 404 -> 380)
+#pragma unroll 2
+            for (int i = 0; i < cnt; ++i) particle(i);
+        } else {
+            for (int i = 0; i < cnt; ++i) particle(i);
         }
     }
     __syncwarp();
