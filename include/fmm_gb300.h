@@ -337,12 +337,13 @@ int fmm_direct(int64_t n, const double* x, const double* y, const double* z,
  * front, or that cannot afford the device-wide synchronisation which
  * cudaMalloc/cudaFree may cause in the middle of a time step.
  *
- * fmm_evaluate_noalloc runs the kernels that fmm_evaluate runs for a plan
- * with {p, basis, FMM_FP64, uniform octree of depth `depth`}, in the same
- * order, and its results agree with that plan's to within 1e-12 relative;
+ * fmm_evaluate_noalloc evaluates a plan with {p, basis, FMM_FP64, uniform
+ * octree of depth `depth`}, the operators in fmm_evaluate's order (the near
+ * field always from both sides of a pair, see fmm_p2p), and its results agree
+ * with that plan's to within 1e-12 relative;
  * but it allocates nothing: no cudaMalloc, no cudaFree, no allocating
  * library routine.  Its working memory (sorted particles, leaf
- * ranges, tree-build counters, expansions, translation matrices, tables) is
+ * ranges, tree-build counters, expansions, folded multipoles, tables) is
  * one fixed __device__ array of FMM_NOALLOC_BYTES_APPROX bytes that every GPU
  * which loads this library holds until the process exits.  Limits:
  * 0 <= n <= FMM_NOALLOC_MAX_N, 0 <= p <= FMM_NOALLOC_MAX_P,
@@ -352,8 +353,8 @@ int fmm_direct(int64_t n, const double* x, const double* y, const double* z,
  *
  * The first call on a device does the set-up (uploads constant tables into
  * the array; synchronous), and a call whose (p, basis) differs from the
- * previous call's on that device rebuilds the translation matrices and the
- * D-tensor table held in the array (synchronous).  Make the first call
+ * previous call's on that device rebuilds the D-tensor table held in the
+ * array (synchronous).  Make the first call
  * before any stream capture.  A call that needs the set-up or a rebuild
  * while its stream is being captured returns FMM_ERR_STATE and queues
  * nothing.  The array's device address is looked up on every call, and a
@@ -365,7 +366,7 @@ int fmm_direct(int64_t n, const double* x, const double* y, const double* z,
 #define FMM_NOALLOC_MAX_N 65536
 #define FMM_NOALLOC_MAX_DEPTH 3
 #define FMM_NOALLOC_MAX_P 6
-#define FMM_NOALLOC_BYTES_APPROX 7540000
+#define FMM_NOALLOC_BYTES_APPROX 7060000
 int fmm_evaluate_noalloc(int p, int basis, int depth, int64_t n, const double* x, const double* y,
                          const double* z, const double* q, double* pot, double* ax, double* ay,
                          double* az, void* stream);

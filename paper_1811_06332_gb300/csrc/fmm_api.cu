@@ -101,7 +101,7 @@ static bool m32_current(const fmm_plan* pl) { return !pl->ad && pl->M32 && pl->W
 // Uniform FP32 and tensor-core plans with the FP32 level shifts keep their
 // local expansions in FP32 only (L32): M2L writes them, L2L updates them and
 // L2P reads them without a conversion to or from FP64 (an FP64 operation
-// holds this part's narrow FP64 pipe for 16 cycles per warp).  L32 is
+// holds this part's narrow FP64 pipe for 17 cycles per warp).  L32 is
 // allocated exactly when these conditions hold.
 static float* L32lev(fmm_plan* pl, int l) { return pl->L32 ? pl->L32 + pl->lvl_off[l] : nullptr; }
 
@@ -655,14 +655,16 @@ int fmm_create(const fmm_config* cfg, fmm_plan** out) {
         *out = pl;
         return FMM_OK;
     }
+    // dense translation matrices: packed for the FP32 shifts, and for FP64 above
+    // the orders that have register kernels
     std::vector<double> W, V;
-    build_translation(cfg->p, bM(pl), W, V);
-    if (cfg->basis == FMM_BASIS_TG) {
+    if (cfg->prec != FMM_FP64 || cfg->p > US_PMAX) build_translation(cfg->p, bM(pl), W, V);
+    if (cfg->basis == FMM_BASIS_TG && cfg->p > US_PMAX) {
         std::vector<double> W1;
         build_translation(cfg->p, 1, W1, V);   // L2L on traceless locals
     }
     const size_t mb = W.size() * sizeof(double), vb = V.size() * sizeof(double);
-    if (cudaMalloc(&pl->W, mb) != cudaSuccess || cudaMalloc(&pl->V, vb) != cudaSuccess ||
+    if ((mb && (cudaMalloc(&pl->W, mb) != cudaSuccess || cudaMalloc(&pl->V, vb) != cudaSuccess)) ||
         cudaMalloc(&pl->Dtab, (size_t)343 * pl->ns * sizeof(double)) != cudaSuccess) {
         fmm_destroy(pl);
         return fail_plan(nullptr, FMM_ERR_OOM, "allocating operator matrices failed");
@@ -676,8 +678,8 @@ int fmm_create(const fmm_config* cfg, fmm_plan** out) {
         offs[3 * o + 2] = near ? 10.0 : rz;
     }
     double* doffs = nullptr;
-    bool ok = cudaMemcpy(pl->W, W.data(), mb, cudaMemcpyHostToDevice) == cudaSuccess &&
-              cudaMemcpy(pl->V, V.data(), vb, cudaMemcpyHostToDevice) == cudaSuccess &&
+    bool ok = (!mb || (cudaMemcpy(pl->W, W.data(), mb, cudaMemcpyHostToDevice) == cudaSuccess &&
+                       cudaMemcpy(pl->V, V.data(), vb, cudaMemcpyHostToDevice) == cudaSuccess)) &&
               cudaMalloc(&doffs, offs.size() * sizeof(double)) == cudaSuccess &&
               cudaMemcpy(doffs, offs.data(), offs.size() * sizeof(double), cudaMemcpyHostToDevice) == cudaSuccess;
     if (ok) {

@@ -80,6 +80,7 @@ int launch_m2m_fused(int p, int64_t n, const double* Mc, const double* delta, do
 int m2m_fused_terms(int p);
 int launch_direct(int64_t n, const double* x, const double* y, const double* z, const double* q, int64_t nt,
                   const int64_t* targets, double* pot, double* ax, double* ay, double* az, cudaStream_t s);
+constexpr int US_PMAX = 8;   // FP64 level shifts in registers up to this order (W, V unused)
 int launch_m2m_level(int p, int basis, int l, const double* W, const double* Mch, int64_t nch, double* Mpa,
                      int64_t npa, cudaStream_t s);
 int launch_l2l_level(int p, int basis, int l, const double* V, const double* Lpa, int64_t npa, double* Lch,

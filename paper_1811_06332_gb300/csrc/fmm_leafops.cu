@@ -38,7 +38,7 @@ k_p2m_leaf(int basis, int depth, int64_t nleaf, const int* __restrict__ start, c
     if (c >= nleaf) return;
     // the leaf centre in FP64 only for the FP64 coordinates; the FP32 path
     // scales by the exact power of two in FP32 (an FP64 operation costs a
-    // warp 16 cycles of this part's narrow FP64 pipe)
+    // warp 17 cycles of this part's narrow FP64 pipe)
     const float inv_hf = (float)(1 << depth);
     double inv_h = 0.0, cx = 0.0, cy = 0.0, cz = 0.0;
     if (!pos32) {

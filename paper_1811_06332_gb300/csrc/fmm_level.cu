@@ -93,7 +93,6 @@ k_l2l_level(int p, int basis, int l, const double* __restrict__ V, const double*
     int launch_ul2l_p##P(int basis, int l, const double* Lpa, int64_t npa, double* Lch, int64_t nch, cudaStream_t s);
 US_DECL(0) US_DECL(1) US_DECL(2) US_DECL(3) US_DECL(4) US_DECL(5) US_DECL(6) US_DECL(7) US_DECL(8)
 #undef US_DECL
-constexpr int US_PMAX = 8;
 
 int launch_m2m_level(int p, int basis, int l, const double* W, const double* Mch, int64_t nch, double* Mpa,
                      int64_t npa, cudaStream_t s) {

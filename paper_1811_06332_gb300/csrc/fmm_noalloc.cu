@@ -1,8 +1,8 @@
 // fmm_evaluate_noalloc: the FP64 uniform-octree FMM for callers that must
 // not allocate device memory.  Every buffer the evaluation needs (sorted
-// particles, leaf ranges, tree-build counters, expansions, translation
-// matrices, D-tensor table, combinatorial tables) lives in one file-scope
-// __device__ array of fixed size; nothing is allocated on any call.
+// particles, leaf ranges, tree-build counters, expansions, folded multipoles,
+// D-tensor table, combinatorial tables) lives in one file-scope __device__
+// array of fixed size; nothing is allocated on any call.
 #include <cstring>
 #include <string>
 #include <vector>
@@ -32,7 +32,7 @@ constexpr int64_t O_DTAB = O_OFFS + al(343 * 3 * 8);
 // cells per component and level), and partial sums of seven shares of the orbits
 constexpr int NA_SHARES = 7;
 constexpr int64_t O_F = O_DTAB + al(343 * NA_NC * 8);
-constexpr int64_t NA_PART = NA_SHARES * NA_NC * (64 + 512) + 60288;   // doubles; the rest keeps the array at its stated size
+constexpr int64_t NA_PART = NA_SHARES * NA_NC * (64 + 512);   // doubles
 constexpr int64_t O_PART = O_F + al((NA_MAX_P + 1) * (NA_MAX_P + 1) * (64 + 32 + 512 + 32) * 8);
 constexpr int64_t O_XS = O_PART + al(NA_PART * 8);
 constexpr int64_t O_PERM = O_XS + al(4 * NA_MAX_N * 8);
@@ -52,7 +52,7 @@ static __device__ __align__(256) unsigned char g_noalloc_scratch[NA_BYTES];
 
 struct NaState {
     unsigned char* base = nullptr;  // device address of g_noalloc_scratch whose tables are uploaded
-    int p = -1, basis = -1;         // translation matrices currently held
+    int p = -1, basis = -1;         // of the last call (the D-tensor table is for this p)
 };
 NaState g_na[64];
 
@@ -160,7 +160,8 @@ extern "C" int fmm_evaluate_noalloc(int p, int basis, int depth, int64_t n, cons
     double* Lb = (double*)(b + O_L);
     int64_t lo[NA_MAX_DEPTH + 1], tot = 0;
     for (int l = 0; l <= depth; ++l) { lo[l] = tot; tot += (int64_t)nc << (3 * l); }
-    // the kernels fmm_evaluate runs for an FMM_FP64 uniform plan, in its order
+    // the kernels of an FMM_FP64 uniform plan in fmm_evaluate's order; the near field
+    // always in its one-sided form (no room for the mutual form's slots)
     if (launch_uniform_tree(n, depth, x, y, z, q, xs, ys, zs, qs, perm, start, b + O_TREE, s) != 0)
         return na_fail(FMM_ERR_CUDA, "tree build failed", cudaGetLastError());
     launch_p2m_leaf(0, p, basis, depth, nleaf, start, xs, ys, zs, qs, Mb + lo[depth], T, s);
