@@ -501,12 +501,12 @@ int fmm_direct(int64_t n, const double* x, const double* y, const double* z, con
 // plan
 // ---------------------------------------------------------------------------
 static void free_tree(fmm_plan* pl) {
-    // the captured step holds the addresses of the buffers freed here
-    if (pl->ugexec) { cudaGraphExecDestroy(pl->ugexec); pl->ugexec = nullptr; }
     cudaFree(pl->xs); cudaFree(pl->ys); cudaFree(pl->zs); cudaFree(pl->qs);
     cudaFree(pl->perm); cudaFree(pl->start); cudaFree(pl->scratch);
     cudaFree(pl->Mbuf); cudaFree(pl->Lbuf); cudaFree(pl->M32); cudaFree(pl->Mbf); cudaFree(pl->pos32);
     cudaFree(pl->dip); cudaFree(pl->msym32); cudaFree(pl->L32); cudaFree(pl->mfold); cudaFree(pl->mpart); cudaFree(pl->pslots); cudaFree(pl->pos32c);
+    // the captured step holds the addresses of these buffers (freeing them has waited for it)
+    if (pl->ugexec) { cudaGraphExecDestroy(pl->ugexec); pl->ugexec = nullptr; }
     pl->pos32c = nullptr;
     pl->msym32 = nullptr;
     pl->L32 = nullptr;
