@@ -120,31 +120,59 @@ k_rf_fold(int sym, int nc, int nt, int lo, int hi, const TI* __restrict__ M, T* 
     F[(int64_t)t * (ncell + RF_PAD_CELLS) + i] = v;
 }
 
-// Partial sums of the split levels, added in group order; FP32 sums carry their
-// rounding errors along (the exact error of each addition), so that the result
-// is rounded once whatever the number of shares.
+// one more share's partial sum onto s; FP32: its rounding error, exact, onto c
+template <typename OT>
+__device__ __forceinline__ void rf_add(OT a, OT& s, OT& c) {
+    const OT t = s + a;
+    if constexpr (sizeof(OT) == 4) {
+        const OT u = t - s;
+        c += (s - (t - u)) + (a - u);
+    }
+    s = t;
+}
+
+// Partial sums of the split levels, in a fixed order; FP32 sums carry their
+// rounding errors along, so that the result is rounded once whatever the number
+// of shares.  Levels of more than RF_FEW shares have few cells: there the first
+// `deep` blocks take 32 components each, a warp every eighth share (a thread
+// alone would wait for 56 loads in turn; loads unrolled in flight took longer
+// still, for the instructions' own fetches: depth 2, p = 3, 18 and 27 us; so 6.5).
+constexpr int RF_FEW = 8;
 template <typename OT>
 __global__ void __launch_bounds__(256)
-k_rf_sum(RfLevels lv, int nrow, const OT* __restrict__ part, OT* __restrict__ Lt) {
-    int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x;
-    for (int k = 0; k < lv.n; ++k) {
-        const RfLevel& v = lv.v[k];
-        if (v.g == 1) continue;
-        const int64_t m = (int64_t)nrow << (3 * v.l);
-        if (i >= m) { i -= m; continue; }
-        const OT* p = part + v.part + i;
-        OT s = p[0], c = OT(0);
-        for (int g = 1; g < v.g; ++g) {
-            const OT a = p[(int64_t)g * m], t = s + a;
-            if constexpr (sizeof(OT) == 4) {
-                const OT u = t - s;
-                c += (s - (t - u)) + (a - u);
-            }
-            s = t;
-        }
-        Lt[v.L + i] = s + c;
-        return;
+k_rf_sum(RfLevels lv, int nrow, int deep, const OT* __restrict__ part, OT* __restrict__ Lt) {
+    __shared__ OT sS[8][32], sC[8][32];
+    const bool many = (int)blockIdx.x < deep;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    int64_t i = many ? (int64_t)blockIdx.x * 32 + lane : (int64_t)(blockIdx.x - deep) * 256 + threadIdx.x;
+    int k = 0;
+    for (; k < lv.n; ++k) {
+        const int g = lv.v[k].g;
+        if (many ? g <= RF_FEW : g == 1 || g > RF_FEW) continue;
+        const int64_t m = (int64_t)nrow << (3 * lv.v[k].l);
+        if (i < m) break;
+        i -= m;
     }
+    if (k >= lv.n) return;   // many: the components are a multiple of 32, so never
+    const RfLevel& v = lv.v[k];
+    const int64_t m = (int64_t)nrow << (3 * v.l);
+    const OT* p = part + v.part + i;
+    OT s = OT(0), c = OT(0);
+    const int step = many ? 8 : 1;
+#pragma unroll 1
+    for (int g = many ? w : 0; g < v.g; g += step) rf_add(p[g * m], s, c);
+    if (many) {
+        sS[w][lane] = s;
+        sC[w][lane] = c;
+        __syncthreads();
+        if (w) return;
+#pragma unroll 1
+        for (int g = 1; g < 8; ++g) {
+            rf_add(sS[g][lane], s, c);
+            c += sC[g][lane];
+        }
+    }
+    Lt[v.L + i] = s + c;
 }
 
 // M2L of the uniform levels lo..hi of a plan whose levels 2..deep run here.
@@ -161,10 +189,10 @@ int launch_m2l_reflect(int out, int p, int symM, int symL, int lo, int hi, int d
     const int nt = nt_of(p), ncM = symM ? ns_of(p) : nt, nrow = symL ? ns_of(p) : nt;
     RfLevels lv;
     const int units = rf_levels(nrow, lo, hi, deep, lvl_off, p, rf_sms(), most, out != 0, lv);
-    int64_t cells = 0, sums = 0;
+    int64_t cells = 0, many = 0, few = 0;   // components summed over many shares, over few
     for (int l = lo; l <= hi; ++l) cells += ((int64_t)1 << (3 * l)) + RF_PAD_CELLS;
     for (int i = 0; i < lv.n; ++i)
-        if (lv.v[i].g > 1) sums += (int64_t)nrow << (3 * lv.v[i].l);
+        if (lv.v[i].g > 1) (lv.v[i].g > RF_FEW ? many : few) += (int64_t)nrow << (3 * lv.v[i].l);
     const dim3 gf((unsigned)((cells + 255) / 256), (unsigned)nt);
     if (out == 0) k_rf_fold<double, double><<<gf, 256, 0, s>>>(symM, ncM, nt, lo, hi, M, (double*)F);
     else if (M32) k_rf_fold<float, float><<<gf, 256, 0, s>>>(symM, ncM, nt, lo, hi, M32, (float*)F);
@@ -175,10 +203,10 @@ int launch_m2l_reflect(int out, int p, int symM, int symL, int lo, int hi, int d
                                           RF_ROW(6), RF_ROW(7), RF_ROW(8), RF_ROW(9), RF_ROW(10)};
 #undef RF_ROW
     int n = 1 + f[p][out](lv, F, Dtab, Lt, part, symL, nrow, (units + 3) / 4, s);
-    if (sums > 0) {
-        const unsigned g = (unsigned)((sums + 255) / 256);
-        if (out == 2) k_rf_sum<float><<<g, 256, 0, s>>>(lv, nrow, (const float*)part, (float*)Lt);
-        else k_rf_sum<double><<<g, 256, 0, s>>>(lv, nrow, (const double*)part, (double*)Lt);
+    if (many + few > 0) {
+        const unsigned deep = (unsigned)(many / 32), g = deep + (unsigned)((few + 255) / 256);
+        if (out == 2) k_rf_sum<float><<<g, 256, 0, s>>>(lv, nrow, (int)deep, (const float*)part, (float*)Lt);
+        else k_rf_sum<double><<<g, 256, 0, s>>>(lv, nrow, (int)deep, (const double*)part, (double*)Lt);
         ++n;
     }
     return n;
