@@ -133,11 +133,12 @@ __device__ __forceinline__ void rf_add(OT a, OT& s, OT& c) {
 
 // Partial sums of the split levels, in a fixed order; FP32 sums carry their
 // rounding errors along, so that the result is rounded once whatever the number
-// of shares.  Levels of more than RF_FEW shares have few cells: there the first
-// `deep` blocks take 32 components each, a warp every eighth share (a thread
+// of shares.  Where levels of up to 512 cells have more than RF_FEW shares, the
+// first `deep` blocks take 32 components each, a warp every eighth share (a thread
 // alone would wait for 56 loads in turn; loads unrolled in flight took longer
 // still, for the instructions' own fetches: depth 2, p = 3, 18 and 27 us; so 6.5).
 constexpr int RF_FEW = 8;
+__host__ __device__ __forceinline__ bool rf_many(const RfLevel& v) { return v.l <= 3 && v.g > RF_FEW; }
 template <typename OT>
 __global__ void __launch_bounds__(256)
 k_rf_sum(RfLevels lv, int nrow, int deep, const OT* __restrict__ part, OT* __restrict__ Lt) {
@@ -147,8 +148,7 @@ k_rf_sum(RfLevels lv, int nrow, int deep, const OT* __restrict__ part, OT* __res
     int64_t i = many ? (int64_t)blockIdx.x * 32 + lane : (int64_t)(blockIdx.x - deep) * 256 + threadIdx.x;
     int k = 0;
     for (; k < lv.n; ++k) {
-        const int g = lv.v[k].g;
-        if (many ? g <= RF_FEW : g == 1 || g > RF_FEW) continue;
+        if (rf_many(lv.v[k]) != many || lv.v[k].g == 1) continue;
         const int64_t m = (int64_t)nrow << (3 * lv.v[k].l);
         if (i < m) break;
         i -= m;
@@ -158,10 +158,12 @@ k_rf_sum(RfLevels lv, int nrow, int deep, const OT* __restrict__ part, OT* __res
     const int64_t m = (int64_t)nrow << (3 * v.l);
     const OT* p = part + v.part + i;
     OT s = OT(0), c = OT(0);
-    const int step = many ? 8 : 1;
+    if (!many) {
+#pragma unroll 4
+        for (int g = 0; g < v.g; ++g) rf_add(p[g * m], s, c);
+    } else {
 #pragma unroll 1
-    for (int g = many ? w : 0; g < v.g; g += step) rf_add(p[g * m], s, c);
-    if (many) {
+        for (int g = w; g < v.g; g += 8) rf_add(p[g * m], s, c);
         sS[w][lane] = s;
         sC[w][lane] = c;
         __syncthreads();
@@ -192,7 +194,7 @@ int launch_m2l_reflect(int out, int p, int symM, int symL, int lo, int hi, int d
     int64_t cells = 0, many = 0, few = 0;   // components summed over many shares, over few
     for (int l = lo; l <= hi; ++l) cells += ((int64_t)1 << (3 * l)) + RF_PAD_CELLS;
     for (int i = 0; i < lv.n; ++i)
-        if (lv.v[i].g > 1) (lv.v[i].g > RF_FEW ? many : few) += (int64_t)nrow << (3 * lv.v[i].l);
+        if (lv.v[i].g > 1) (rf_many(lv.v[i]) ? many : few) += (int64_t)nrow << (3 * lv.v[i].l);
     const dim3 gf((unsigned)((cells + 255) / 256), (unsigned)nt);
     if (out == 0) k_rf_fold<double, double><<<gf, 256, 0, s>>>(symM, ncM, nt, lo, hi, M, (double*)F);
     else if (M32) k_rf_fold<float, float><<<gf, 256, 0, s>>>(symM, ncM, nt, lo, hi, M32, (float*)F);
